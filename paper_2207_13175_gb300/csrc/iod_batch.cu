@@ -52,7 +52,7 @@ struct SlotH {
 
 // per-slot allocation layout (every region 256-byte aligned)
 struct Layout {
-    size_t obs, ep, rc64, misc, swarm, blk, trace, mix, cs, od, ct, lm, budget, total;
+    size_t obs, ep, rc64, misc, swarm, blk, trace, mix, cs, od, ct, lm, total;
 };
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -88,11 +88,8 @@ Layout layout(int K, int m, int n_tiles, int trace_cap, long long steps_bound, b
         L.lm = o;
         o = up256(o + sizeof(double) * (kLmVecs * 2 * (size_t)K + kLmTail));
     }
-    L.budget = o;
     // the split residuals' table and, for small swarms and refinements, the chief's positions
-    // by FP64 steps: about a hundred bytes per epoch beside the swarm's 160 per particle.
-    // They are allocated with the rest but not held against the caller's budget, which
-    // admits the same requests with or without them.
+    // by FP64 steps
     L.ep = o;
     o = up256(o + kEpochBytes * (size_t)K);
     if (m < kFp64Swarm || refine) {
@@ -174,7 +171,7 @@ struct iod_batch {
     {
         const int nt = (r.m + cls_block[class_of(r.m)] - 1) / cls_block[class_of(r.m)];
         return layout((int)r.t.size(), r.m, nt, trace_cap_for(r), steps_bound(r.t, dt_of(r.m)), mixed(),
-                      opt.refine_iters > 0).budget;
+                      opt.refine_iters > 0).total;
     }
 
     void drop_graph()
@@ -243,7 +240,7 @@ int admit(iod_batch *b)
             r.state = kFailed;     // nothing resident whose memory could come back
             continue;
         }
-        S.bytes = L.budget;
+        S.bytes = L.total;
         S.smem_mix = b->mixed() ? mixed_smem_bytes(K, S.steps_bound) : 0;
         S.smem_fp64 = swarm_smem_bytes(K, IOD_RK4);
         S.cost = (double)S.steps_bound;
@@ -362,7 +359,7 @@ int admit(iod_batch *b)
         r.state = kResident;
         r.slot = si;
         r.t_admit = b->now();
-        b->in_use += L.budget;
+        b->in_use += L.total;
         b->high_water = std::max(b->high_water, b->in_use);
         ids.push_back(si);
         b->dirty = true;
