@@ -179,36 +179,31 @@ struct Fp64Step {
     bool near;
 };
 
-__device__ __forceinline__ void fp64_bits(const ff::State &s, double d[6])
-{
-    double r[9];
-    ff::pack_state(s, r);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) d[q] = r[q];
-}
-
 __device__ __noinline__ Fp64Step fp64_step(Dyn D, double h, float2 rmin, ff::State s, bool bits)
 {
     double d[6];
     if (bits)
-        fp64_bits(s, d);
+        ff::held_fp64(s, d);
     else
         ff::from_state(D.omu, s, d);
     rk4_step(D, rk_h(h), d);
     const float x = (float)(d[0] - D.omu), y = (float)d[1], z = (float)d[2];
     const float u = (float)d[3], v = (float)d[4], w = (float)d[5];
     const float rm = fmaf(x, x, fmaf(y, y, z * z));
-    if (ff::step_ok(rmin, make_float2(rm + fmaf(2.0f, x, 1.0f), rm), fmaf(u, u, fmaf(v, v, w * w))))
-        return Fp64Step{ff::to_state(D.omu, d), false};
-    const double r[9] = {d[0], d[1], d[2], d[3], d[4], d[5], 0.0, 0.0, 0.0};
-    return Fp64Step{ff::unpack_state(r), true};
+    if (ff::step_ok(rmin, make_float2(rm + fmaf(2.0f, x, 1.0f), rm), fmaf(u, u, fmaf(v, v, w * w)))) {
+        const ff::State S = ff::to_state(D.omu, d);
+        return Fp64Step{S, ff::holds_fp64(S)};
+    }
+    return Fp64Step{ff::hold_fp64(d, 0u), true};
 }
 
 // n steps of size h of the circular problem on a split state (iod_ff.cuh): split steps
 // where they are at least as exact as FP64 ones, else FP64 steps, decided lane by lane from
 // the state alone, so the result does not depend on which lanes run together.  The
-// attraction that a split step passes on to the next is formed anew at the start.
-__device__ __forceinline__ void rk4_interval(const Dyn &D, const ff::Mass &M, double h, int n, ff::State &s)
+// attraction that a split step passes on to the next is formed anew at the start.  held:
+// whether s holds FP64 values (ff::holds_fp64), on entry and on return.
+__device__ __forceinline__ void rk4_interval(const Dyn &D, const ff::Mass &M, double h, int n, ff::State &s,
+                                             bool &held)
 {
     if (n <= 0) return;
     const float hf = (float)h;
@@ -219,7 +214,7 @@ __device__ __forceinline__ void rk4_interval(const Dyn &D, const ff::Mass &M, do
     ff::Grav G;
     float2 r2;
     int taken = 0;
-    bool bits = false;       // the FP64 state rides in s
+    bool bits = held;        // the FP64 state rides in s
     bool anew = true;        // the attraction at s is still to be formed
     for (int j = 0; j < n; ++j) {
         if (anew && !bits) ff::attraction(M, s.ph, s.pl, s.zh, s.zl, G, r2);
@@ -236,9 +231,11 @@ __device__ __forceinline__ void rk4_interval(const Dyn &D, const ff::Mass &M, do
     }
     if (bits) {
         double d[6];
-        fp64_bits(s, d);
+        ff::held_fp64(s, d);
         s = ff::to_state(D.omu, d);
+        bits = ff::holds_fp64(s);
     }
+    held = bits;
     if (taken) ff::make_up(M, s, G, (float)taken * (float)(rest - (double)hl));
 }
 
@@ -248,7 +245,7 @@ __device__ __forceinline__ void rk4_interval(const Dyn &D, const ff::Mass &M, do
 // copy was scheduled with twice the dependency stalls (256 particles, 247 steps and 20
 // epochs: 203 us an iteration; inlined 168).
 __device__ __forceinline__ ff::QuadState rk4_interval_quad(const Dyn &D, const ff::Mass &M, const ff::QuadLane &Q,
-                                                           double h, int n, ff::QuadState s)
+                                                           double h, int n, ff::QuadState s, bool &held)
 {
     constexpr unsigned int kAll = 0xffffffffu;
     if (n <= 0) return s;
@@ -260,7 +257,7 @@ __device__ __forceinline__ ff::QuadState rk4_interval_quad(const Dyn &D, const f
     ff::QuadPull G{0.0f, 0.0f};
     float2 r2 = make_float2(0.0f, 0.0f);
     int taken = 0;
-    bool bits = false, anew = true;        // as in rk4_interval
+    bool bits = held, anew = true;        // as in rk4_interval
     for (int j = 0; j < n; ++j) {
         const bool form = anew && !bits;
         if (__any_sync(kAll, form)) {
@@ -301,10 +298,13 @@ __device__ __forceinline__ ff::QuadState rk4_interval_quad(const Dyn &D, const f
         const ff::State S = ff::quad_whole(s);
         if (bits) {
             double d[6];
-            fp64_bits(S, d);
-            s = ff::quad_part(Q, ff::to_state(D.omu, d));
+            ff::held_fp64(S, d);
+            const ff::State T = ff::to_state(D.omu, d);
+            s = ff::quad_part(Q, T);
+            bits = ff::holds_fp64(T);
         }
     }
+    held = bits;
     ff::quad_make_up(Q, s, G, (float)taken * (float)(rest - (double)hl), taken != 0);
     return s;
 }
@@ -577,18 +577,13 @@ __device__ __forceinline__ void add_epoch_cost(const CostW &W, double rx, double
 }
 
 // The same from the split residuals (iod_ff_cost.cuh) of the line of sight (h + l for x and
-// y, zh + zl); the FP64 form where those do not apply.
-__device__ __forceinline__ void add_epoch_cost_split(const CostW &W, const ff::Epoch &E, float2 h, float2 l, float zh,
-                                                     float zl, double ra_obs, double dec_obs, double rng_obs,
-                                                     double &J)
+// y, zh + zl); false, and J unchanged, where those do not apply and the FP64 form decides.
+__device__ __forceinline__ bool add_epoch_cost_split(const CostW &W, const ff::Epoch &E, float2 h, float2 l, float zh,
+                                                     float zl, double rng_obs, double &J)
 {
     float2 bh, bl;
     float rh, rl;
-    if (!ff::residuals(E, h, l, zh, zl, bh, bl, rh, rl)) {
-        add_epoch_cost(W, (double)h.x + (double)l.x, (double)h.y + (double)l.y, (double)zh + (double)zl, ra_obs,
-                       dec_obs, rng_obs, J);
-        return;
-    }
+    if (!ff::residuals(E, h, l, zh, zl, bh, bl, rh, rl)) return false;
     const double b_ra = (double)bh.x + (double)bl.x, b_dec = (double)bh.y + (double)bl.y;
     double Jk = fma(b_ra * W.w_ra, b_ra, b_dec * W.w_dec * b_dec);
     if (W.use_range) {
@@ -598,6 +593,7 @@ __device__ __forceinline__ void add_epoch_cost_split(const CostW &W, const ff::E
         Jk = fma(b_rng * W.w_rng, b_rng, Jk);
     }
     J += W.quartic ? Jk * Jk : Jk;
+    return true;
 }
 
 // From an FP64 position (the elliptic problem's and DOPRI5's states); ep null: the FP64
@@ -605,14 +601,13 @@ __device__ __forceinline__ void add_epoch_cost_split(const CostW &W, const ff::E
 __device__ __forceinline__ void add_epoch_cost_any(const CostW &W, const ff::Epoch *ep, int k, double rx, double ry,
                                                    double rz, double ra_obs, double dec_obs, double rng_obs, double &J)
 {
-    if (!ep) {
-        add_epoch_cost(W, rx, ry, rz, ra_obs, dec_obs, rng_obs, J);
-        return;
+    if (ep) {
+        const float2 h = make_float2((float)rx, (float)ry);
+        const float2 l = make_float2((float)(rx - (double)h.x), (float)(ry - (double)h.y));
+        const float zh = (float)rz;
+        if (add_epoch_cost_split(W, ep[k], h, l, zh, (float)(rz - (double)zh), rng_obs, J)) return;
     }
-    const float2 h = make_float2((float)rx, (float)ry);
-    const float2 l = make_float2((float)(rx - (double)h.x), (float)(ry - (double)h.y));
-    const float zh = (float)rz;
-    add_epoch_cost_split(W, ep[k], h, l, zh, (float)(rz - (double)zh), ra_obs, dec_obs, rng_obs, J);
+    add_epoch_cost(W, rx, ry, rz, ra_obs, dec_obs, rng_obs, J);
 }
 
 // ---------------------------------------------------------------------------------

@@ -20,7 +20,8 @@ namespace iod {
 namespace ff {
 
 // One epoch: sines and cosines of the observed angles, and the chief's position as the
-// split step carries it (three words; x from the Moon).  ok = 0: the observed elevation
+// split step carries it (three words; x from the Moon; NaN where it holds FP64 values
+// instead: the FP64 form decides there).  ok = 0: the observed elevation
 // lies outside [-pi/2, pi/2], where the difference of Eq. 8 is not that angle.
 struct alignas(16) Epoch {
     float2 ka, kal;        // (cos a~, sin a~): leading and low words

@@ -9,6 +9,7 @@
 #define IOD_HD __device__ __forceinline__
 #else
 #include <math.h>
+#include <string.h>
 #define IOD_HD static inline
 struct float2 {
     float x, y;
@@ -33,6 +34,12 @@ IOD_HD float rsqrt_est(float x)
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// bits of a value
+IOD_HD unsigned int bits_of(float a) { return __float_as_uint(a); }
+IOD_HD float float_of(unsigned int b) { return __uint_as_float(b); }
+IOD_HD unsigned int high_word(double d) { return (unsigned int)__double2hiint(d); }
+IOD_HD unsigned int low_word(double d) { return (unsigned int)__double2loint(d); }
+IOD_HD double from_halves(unsigned int hi, unsigned int lo) { return __hiloint2double((int)hi, (int)lo); }
 #else
 IOD_HD float add(float a, float b) { return a + b; }
 IOD_HD float sub(float a, float b) { return a - b; }
@@ -42,6 +49,33 @@ IOD_HD float2 add2(float2 a, float2 b) { return float2{a.x + b.x, a.y + b.y}; }
 IOD_HD float2 mul2(float2 a, float2 b) { return float2{a.x * b.x, a.y * b.y}; }
 IOD_HD float2 fma2(float2 a, float2 b, float2 c) { return float2{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
 IOD_HD float rsqrt_est(float x) { return IOD_RSQRT_EST(x); }
+IOD_HD unsigned int bits_of(float a)
+{
+    unsigned int b;
+    memcpy(&b, &a, sizeof b);
+    return b;
+}
+IOD_HD float float_of(unsigned int b)
+{
+    float a;
+    memcpy(&a, &b, sizeof a);
+    return a;
+}
+IOD_HD unsigned long long word_of(double d)
+{
+    unsigned long long b;
+    memcpy(&b, &d, sizeof b);
+    return b;
+}
+IOD_HD unsigned int high_word(double d) { return (unsigned int)(word_of(d) >> 32); }
+IOD_HD unsigned int low_word(double d) { return (unsigned int)word_of(d); }
+IOD_HD double from_halves(unsigned int hi, unsigned int lo)
+{
+    const unsigned long long b = ((unsigned long long)hi << 32) | lo;
+    double d;
+    memcpy(&d, &b, sizeof d);
+    return d;
+}
 #endif
 
 IOD_HD float2 mk2(float a, float b)

@@ -96,9 +96,18 @@ template <int ER>
 struct RkState {
     static constexpr int kRows = 9;
     ff::State S;
-    __device__ __forceinline__ void begin(const Dyn &D, const double x[6]) { S = ff::to_state(D.omu, x); }
+    bool held;               // S holds FP64 values (ff::holds_fp64)
+    __device__ __forceinline__ void begin(const Dyn &D, const double x[6])
+    {
+        S = ff::to_state(D.omu, x);
+        held = ff::holds_fp64(S);
+    }
     __device__ __forceinline__ void pack(double r[kRows]) const { ff::pack_state(S, r); }
-    __device__ __forceinline__ void unpack(const double r[kRows]) { S = ff::unpack_state(r); }
+    __device__ __forceinline__ void unpack(const double r[kRows])
+    {
+        S = ff::unpack_state(r);
+        held = ff::holds_fp64(S);
+    }
     template <class F>
     __device__ __forceinline__ long long advance(const Dyn &D, const ObsView &O, int ka, int kb, F &&f)
     {
@@ -110,7 +119,7 @@ struct RkState {
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(&O.ep[k]));
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(&O.ep[k].zh));
             }
-            rk4_interval(D, M, O.h[k], n, S);
+            rk4_interval(D, M, O.h[k], n, S, held);
             steps += n;
             f(k, *this);
         }
@@ -122,17 +131,16 @@ struct RkState {
     __device__ __forceinline__ void add_cost(const Dyn &D, const CostW &W, const ObsView &O, int k, double &J) const
     {
         const double rng = W.use_range ? O.rng[k] : 0.0;
-        if (O.ep) {
+        if (O.ep && !held) {
             const ff::Epoch E = O.ep[k];
             float2 h, l;
             float zh, zl;
             ff::sight(E, S, h, l, zh, zl);
-            add_epoch_cost_split(W, E, h, l, zh, zl, O.ra[k], O.dec[k], rng, J);
-        } else {
-            double st[6];
-            get(D, st);
-            add_epoch_cost(W, st[0] - O.rcx[k], st[1] - O.rcy[k], st[2] - O.rcz[k], O.ra[k], O.dec[k], rng, J);
+            if (add_epoch_cost_split(W, E, h, l, zh, zl, rng, J)) return;
         }
+        double st[6];
+        get(D, st);
+        add_epoch_cost(W, st[0] - O.rcx[k], st[1] - O.rcy[k], st[2] - O.rcz[k], O.ra[k], O.dec[k], rng, J);
     }
 };
 
@@ -145,7 +153,8 @@ struct RkQuad {
     __device__ __forceinline__ void begin(const Dyn &D, const double x[6])
     {
         Q = ff::quad_lane(ff::make_mass(D.mu, D.omu));
-        s = ff::quad_part(Q, ff::to_state(D.omu, x));
+        whole.begin(D, x);
+        s = ff::quad_part(Q, whole.S);
     }
     template <class F>
     __device__ __forceinline__ long long advance(const Dyn &D, const ObsView &O, F &&f)
@@ -154,7 +163,7 @@ struct RkQuad {
         long long steps = 0;
         for (int k = 0; k < O.n; ++k) {
             const int n = O.ns[k];
-            s = rk4_interval_quad(D, M, Q, O.h[k], n, s);
+            s = rk4_interval_quad(D, M, Q, O.h[k], n, s, whole.held);
             steps += n;
             whole.S = ff::quad_whole(s);
             f(k, whole);
@@ -917,7 +926,7 @@ __device__ long long setup_body(const KParams &P, double vmax_frac, double sig_r
             store(k, st);
             if (!lead) return;
             ff::Epoch &E = ep[k];       // the chief as the particles are carried
-            E.ph = r.S.ph;
+            E.ph = r.held ? make_float2(CUDART_NAN_F, CUDART_NAN_F) : r.S.ph;
             E.pl = r.S.pl;
             E.pc = r.S.pc;
             E.zh = r.S.zh;
