@@ -7,10 +7,12 @@
 #ifdef __CUDACC__
 #include <cuda_runtime.h>
 #define IOD_HD __device__ __forceinline__
+#define IOD_CALL static __device__ __noinline__
 #else
 #include <math.h>
 #include <string.h>
 #define IOD_HD static inline
+#define IOD_CALL static
 struct float2 {
     float x, y;
 };
@@ -34,6 +36,15 @@ IOD_HD float rsqrt_est(float x)
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// the hardware's x^(2/3) for x >= 0 (limits only)
+IOD_HD float pow23_est(float x)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    r = __fmul_rn(r, 0.6666667f);
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(r));
+    return r;
+}
 // bits of a value
 IOD_HD unsigned int bits_of(float a) { return __float_as_uint(a); }
 IOD_HD float float_of(unsigned int b) { return __uint_as_float(b); }
@@ -49,6 +60,7 @@ IOD_HD float2 add2(float2 a, float2 b) { return float2{a.x + b.x, a.y + b.y}; }
 IOD_HD float2 mul2(float2 a, float2 b) { return float2{a.x * b.x, a.y * b.y}; }
 IOD_HD float2 fma2(float2 a, float2 b, float2 c) { return float2{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
 IOD_HD float rsqrt_est(float x) { return IOD_RSQRT_EST(x); }
+IOD_HD float pow23_est(float x) { return powf(x, 0.6666667f); }
 IOD_HD unsigned int bits_of(float a)
 {
     unsigned int b;

@@ -2560,14 +2560,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) init_kernel(KParams P)
         init_body<INTEG, 0>(P, blockIdx.x, gridDim.x);
 }
 
+// (one block per SM at least, as everywhere here: without that bound the compiler keeps to 128
+// registers, and the quads spill up to 48 of the 150 they need)
 template <int INTEG, int LANES>
-__global__ void __launch_bounds__(kMaxThreads) init_kernel_lanes(KParams P)
+__global__ void __launch_bounds__(kMaxThreads, 1) init_kernel_lanes(KParams P)
 {
     init_body_lanes<INTEG, LANES>(P, blockIdx.x, gridDim.x);
 }
 
 template <int INTEG, int LAGGED, int LANES>
-__global__ void __launch_bounds__(kMaxThreads) iter_kernel_lanes(KParams P)
+__global__ void __launch_bounds__(kMaxThreads, 1) iter_kernel_lanes(KParams P)
 {
     iter_body_lanes<INTEG, LAGGED, LANES>(P, blockIdx.x, gridDim.x);
 }
