@@ -29,9 +29,17 @@ struct alignas(16) Epoch {
     float2 ph, pl, pc;     // chief x, y
     float zh, zl, zc;      // chief z
     int ok;
-    float pad[2];
+    float far2;            // squared length of the line of sight up to which the split residuals are taken
+    float pad;
 };
 static_assert(sizeof(Epoch) == 80, "Epoch layout");
+
+// far2 of an epoch that FP64 propagation reaches in n steps.  The split residuals err by 1.4e-15
+// rad (root mean square, up to 0.1 rad; the FP64 form by 7e-17, growing as the elevation's
+// secant), which the rounding of the positions hides for near deputies only: one rounding of
+// the deputy's and the chief's is 1.4e-15 rad at 1/32 LU, and n steps' at least sqrt(n) times
+// that.
+IOD_HD float far_limit(float n) { return mul(add(1.0f, n), 1.0f / 1024.0f); }
 
 // atan(i / 128), i = 0..128, in two words
 struct AtanTable {
@@ -167,7 +175,8 @@ IOD_HD void sqrt2w(float ah, float al, float &h, float &l)
 // Residual magnitudes of the epoch for the line of sight (x, y packed; z), two words each:
 // ba, bb in two words, and rho_xy.  r2: |rho|^2 (one word).  False where the split form
 // does not apply (a line of sight along the pole or out of FP32's range, an observed
-// elevation beyond the poles): the FP64 form decides there.
+// elevation beyond the poles) or is the less exact one (far2 of the epoch, and less than
+// 83 degrees from the equator): the FP64 form decides there.
 IOD_HD bool residuals(const Epoch &E, float2 h, float2 l, float zh, float zl, float2 &bh, float2 &bl, float &rxyh,
                       float &rxyl)
 {
@@ -176,7 +185,7 @@ IOD_HD bool residuals(const Epoch &E, float2 h, float2 l, float zh, float zl, fl
     two_sum(q.x, q.y, s, se);
     se = add(se, add(qe.x, qe.y));
     const float r2 = ffma(zh, zh, s);
-    if (!(s >= 1e-28f && r2 <= 1e28f) || !E.ok) return false;
+    if (!(s >= 1e-28f && r2 <= 1e28f) || !E.ok || (r2 > E.far2 && mul(64.0f, s) >= r2)) return false;
     sqrt2w(s, se, rxyh, rxyl);
     float2 ah, al, ch, cl;
     turn(E.ka, E.kal, h.x, l.x, h.y, l.y, ah, al);

@@ -872,6 +872,8 @@ __device__ void setup_angles(const KParams &P, ff::Epoch *ep, int tid, int n)
         E.kb = make_float2((float)cb, (float)sb);
         E.kbl = make_float2((float)(cb - (double)E.kb.x), (float)(sb - (double)E.kb.y));
         E.ok = fabs(P.dec[k]) <= 1.5707963267948966;
+        // (DOPRI5 at 1e-12 takes steps of about 1/90; at looser tolerances their own error counts)
+        E.far2 = ff::far_limit((float)(P.integrator == kRK4 ? P.t[k] / P.dt : P.t[k] * 64.0));
     }
 }
 
