@@ -335,8 +335,12 @@ int iod_propagate(iod_problem *p, const double *x0, int m, double *out);
  *   max_iters iterations (each: a central-difference Jacobian and eight damped trials)
  *   form      0: least squares on the weighted angle residuals (2 n_obs entries; the
  *             minimised sum is the CHI2 cost); 1: on the per-epoch b_k^T W b_k (Eq. 15)
- *   x_out     host [6] refined state; cost_out: its sum of squared residuals;
- *   iters_out iterations run.  Synchronising.  IOD_EINVAL for a DOPRI5 problem. */
+ *   x_out     host [6] refined state; cost_out: its sum of squared residuals, by FP64 steps.
+ *             x0 itself, with its cost by iod_eval's evaluation, if no state was found whose
+ *             cost is below that (near a minimum FP64 rounding can put a state first that
+ *             the more exact evaluation does not).  Beside a swarm on FP64 steps (below
+ *             256 particles) FP64 alone decides.
+ *   iters_out iterations run, also when x0 is kept.  Synchronising.  IOD_EINVAL for a DOPRI5 problem. */
 int iod_refine(iod_problem *p, const double x0[6], int max_iters, int form, double x_out[6],
                double *cost_out, int *iters_out);
 

@@ -197,7 +197,7 @@ struct iod_problem {
     }
 
     // the kernels' view of the problem and its swarm; caller = true: for states of the
-    // caller's (evaluation, propagation, refinement), which always take the split step
+    // caller's (evaluation, propagation), which always take the split step
     KParams params(bool caller = false) const
     {
         KParams P{};
@@ -1288,7 +1288,7 @@ int iod_refine(iod_problem *p, const double x0[6], int max_iters, int form, doub
     if (int rc64 = ensure_rc64(p)) return rc64;
     double *R = (double *)p->lm.ptr, *dx0 = R + iod::kLmVecs * (size_t)n + iod::kLmTail, *dout = dx0 + 6;
     IOD_CUDA(cudaMemcpyAsync(dx0, x0, 6 * sizeof(double), cudaMemcpyHostToDevice, p->stream), "cudaMemcpyAsync");
-    cudaError_t e = iod::launch_lm(p->params(true), dx0, max_iters, form, p->sigma[0], p->sigma[1], R, dout, p->stream);
+    cudaError_t e = iod::launch_lm(p->params(), dx0, max_iters, form, p->sigma[0], p->sigma[1], R, dout, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "refinement kernel launch");
     double out[9];
     IOD_CUDA(cudaMemcpyAsync(out, dout, sizeof out, cudaMemcpyDeviceToHost, p->stream), "cudaMemcpyAsync");

@@ -3053,9 +3053,10 @@ struct LmState {
     double A[36], g[6];
 };
 
-// The start: the estimate x0 and its cost; damping 1e-3.
-__device__ void lm_start(const Dyn &D, const ObsView &O, LmState &S, const double *x0, int form, double sig_ra,
-                         double sig_dec, double *R)
+// The start: the estimate x0 and its cost; damping 1e-3.  s0 (null: not needed): its cost by
+// the swarm's split evaluation, formed by the second warp beside the first one's residuals.
+__device__ void lm_start(const KParams &P, const Dyn &D, const ObsView &O, LmState &S, const double *x0, int form,
+                         double sig_ra, double sig_dec, double *R, double *s0)
 {
     const int t = threadIdx.x;
     if (t < 6) S.x[t] = x0[t];
@@ -3072,6 +3073,7 @@ __device__ void lm_start(const Dyn &D, const ObsView &O, LmState &S, const doubl
         S.ctr = 0;
         S.tprev = 3;
     }
+    if (s0 && t == 32) *s0 = lm_split_cost(P, x0, form);
     __syncthreads();
 }
 
@@ -3249,22 +3251,28 @@ __device__ void lm_iterate(const Dyn &D, const ObsView &O, LmState &S, int max_i
     }
 }
 
-// The end of a refinement of x0 (cost c0 of its residuals).  It runs on FP64 steps, which
-// round as the plain FP64 method does; the swarms take the more exact split step, and at
-// the rounding floor of either a state that is better by the one can be worse by the
-// other.  So the result must not be worse than the start by the swarm's evaluation (else the
-// start is kept), and its cost is the lower of its two evaluations.  Block-collective.
-__device__ void lm_close(const KParams &P, LmState &S, const double *x0, double c0, int form)
+// Whether a refinement has to be closed by the swarm's evaluation: it runs on FP64 steps, and so
+// do the small swarms, but the others take the more exact split step.
+__device__ __forceinline__ bool lm_closes(const KParams &P) { return !P.dynamics && !P.fp64; }
+
+// The end of a refinement of x0, whose cost by the swarm's evaluation is s0.  At the rounding
+// floor a state that is better by the one evaluation can be worse by the other, so the
+// refined state has to be better than s0 by its own cost and, where that is not clearly
+// below (the FP64 steps' rounding is far less than a half of any cost but one at its
+// floor), not worse by the swarm's; else the start is kept, with s0 as its cost.  A refined
+// state's cost is the FP64 sum of its squared residuals.  Block-collective.
+__device__ void lm_close(const KParams &P, LmState &S, const double *x0, double s0, int form)
 {
-    __shared__ double s_js[2];
-    if (P.dynamics || S.stop == 2) return;
-    if (threadIdx.x < 2) s_js[threadIdx.x] = lm_split_cost(P, threadIdx.x ? S.x : x0, form);
-    __syncthreads();
+    if (!lm_closes(P) || S.stop == 2) return;
     if (threadIdx.x == 0) {
-        const bool keep = s_js[1] > s_js[0];
-        if (keep)
+        bool keep = true;
+        for (int q = 0; q < 6; ++q) keep = keep && S.x[q] == x0[q];
+        keep = keep || !(S.c <= s0);
+        if (!keep && S.c > 0.5 * s0) keep = lm_split_cost(P, S.x, form) > s0;
+        if (keep) {
             for (int q = 0; q < 6; ++q) S.x[q] = x0[q];
-        S.c = keep ? fmin(c0, s_js[0]) : fmin(S.c, s_js[1]);
+            S.c = s0;
+        }
     }
     __syncthreads();
 }
@@ -3274,10 +3282,10 @@ __device__ void lm_body(const KParams &P, const ObsView &O, const double *x0, in
 {
     const Dyn D = make_dyn(P);
     __shared__ LmState S;
-    lm_start(D, O, S, x0, form, sig_ra, sig_dec, R);
-    const double c0 = S.c;
+    __shared__ double s_s0;
+    lm_start(P, D, O, S, x0, form, sig_ra, sig_dec, R, lm_closes(P) ? &s_s0 : nullptr);
     lm_iterate(D, O, S, max_iters, max_iters, form, sig_ra, sig_dec, R, P.n_obs);
-    lm_close(P, S, x0, c0, form);
+    lm_close(P, S, x0, s_s0, form);
     if (threadIdx.x == 0) {
         for (int q = 0; q < 6; ++q) out[q] = S.x[q];
         out[6] = S.c;
@@ -3302,7 +3310,8 @@ __global__ void __launch_bounds__(128) lm_kernel(KParams P, const double *__rest
 // iterations per action.  The first action keeps the swarm's best (g_pso, gJ_pso) and
 // takes the start; from then on g and gJ hold the current estimate and its cost (the
 // estimate only ever moves to a lower cost, so it stays evaluable), with the damping,
-// iteration count and stop reason beside them.  The last action sets kFlagRefined; a
+// iteration count and stop reason beside them.  The last action closes it against the
+// recorded cost of the swarm's best (lm_close) and sets kFlagRefined; a
 // start that is not evaluable ends at once and keeps the swarm's best.  Returns true in
 // every thread (the action's only tile).
 __device__ bool refine_body(const KParams &P, int max_iters, double sig_ra, double sig_dec, double *R)
@@ -3313,18 +3322,18 @@ __device__ bool refine_body(const KParams &P, int max_iters, double sig_ra, doub
     const int form = P.cost_form == 1 ? 1 : 0;
     GBest *gb = P.gb;
     __shared__ LmState S;
-    __shared__ double s_x0[6], s_p0[6], s_c0;      // the estimate; the refinement's start and its cost
+    __shared__ double s_x0[6], s_p0[6], s_s0;      // the estimate; the refinement's start and its recorded cost
     __shared__ int s_started;
     if (threadIdx.x == 0) s_started = (__ldcg(&gb->flags) & kFlagLmStarted) != 0;
     if (threadIdx.x < 6) s_x0[threadIdx.x] = __ldcg(&gb->g[threadIdx.x]);
     __syncthreads();
     if (!s_started) {
-        lm_start(D, O, S, s_x0, form, sig_ra, sig_dec, R);
+        lm_start(P, D, O, S, s_x0, form, sig_ra, sig_dec, R, nullptr);
         if (threadIdx.x < 6) s_p0[threadIdx.x] = s_x0[threadIdx.x];
         if (threadIdx.x == 0) {
-            s_c0 = S.c;
             for (int q = 0; q < 6; ++q) gb->g_pso[q] = s_x0[q];
-            gb->gJ_pso = __ldcg(&gb->gJ);
+            s_s0 = __ldcg(&gb->gJ);
+            gb->gJ_pso = s_s0;
         }
     } else {
         const int n = form == 0 ? 2 * P.n_obs : P.n_obs;
@@ -3342,12 +3351,12 @@ __device__ bool refine_body(const KParams &P, int max_iters, double sig_ra, doub
             S.col = (int)__ldcg(&tail[43]);
             S.ctr = (int)__ldcg(&tail[44]);
             S.tprev = (int)__ldcg(&tail[45]);
-            s_c0 = __ldcg(&tail[46]);
+            s_s0 = __ldcg(&gb->gJ_pso);
         }
     }
     __syncthreads();
     lm_iterate(D, O, S, max_iters, S.it + kLmItersPerAction, form, sig_ra, sig_dec, R, P.n_obs);
-    if (lm_finished(S, max_iters)) lm_close(P, S, s_p0, s_c0, form);
+    if (lm_finished(S, max_iters)) lm_close(P, S, s_p0, s_s0, form);
     {   // the carried part of the state, for the next action
         const int n = form == 0 ? 2 * P.n_obs : P.n_obs;
         double *tail = R + (size_t)kLmVecs * n;
@@ -3358,7 +3367,6 @@ __device__ bool refine_body(const KParams &P, int max_iters, double sig_ra, doub
             tail[43] = (double)S.col;
             tail[44] = (double)S.ctr;
             tail[45] = (double)S.tprev;
-            tail[46] = s_c0;
         }
     }
     __syncthreads();   // the block's writes before thread 0's fence and flags
