@@ -189,15 +189,17 @@ struct iod_problem {
         return mix_ct_offset() + sizeof(float) * (size_t)((mix_cap + ch - 1) / ch + 1);
     }
 
-    // whether a swarm of n particles keeps the FP64 step (kFp64Swarm)
+    bool fp64_all = false;       // FP64 steps throughout (circular problem, RK4; long_steps)
+
+    // whether a swarm of n particles keeps the FP64 step (kFp64Swarm, kMaxSplitStep)
     bool fp64_steps(int n) const
     {
-        return opt.integrator == IOD_RK4 && opt.dynamics == IOD_CR3BP &&
-               (opt.shard_total > 0 ? opt.shard_total : n) < iod::kFp64Swarm;
+        return fp64_all || (opt.integrator == IOD_RK4 && opt.dynamics == IOD_CR3BP &&
+                            (opt.shard_total > 0 ? opt.shard_total : n) < iod::kFp64Swarm);
     }
 
     // the kernels' view of the problem and its swarm; caller = true: for states of the
-    // caller's (evaluation, propagation), which always take the split step
+    // caller's (evaluation, propagation), which take the split step also beside a small swarm
     KParams params(bool caller = false) const
     {
         KParams P{};
@@ -243,7 +245,7 @@ struct iod_problem {
         P.rc = d_rc();
         P.rc64 = d_rc64();
         P.ep = d_ep();
-        P.fp64 = !caller && m > 0 && fp64_steps(m);
+        P.fp64 = fp64_all || (!caller && m > 0 && fp64_steps(m));
         P.h = d_h();
         P.nsteps = d_ns();
         P.cst = d_cst();
@@ -302,6 +304,20 @@ double er3bp_true_anomaly(double e, double f0, double tau)
         if (std::fabs(dE) <= 1e-15 * std::fmax(1.0, std::fabs(E))) break;
     }
     return E + 2.0 * std::atan(b * std::sin(E) / (1.0 - b * std::cos(E)));
+}
+
+bool long_steps(const double *t, int n, double dt)
+{
+    long long steps = 0, steps_long = 0;
+    for (int k = 0; k < n; ++k) {
+        const double span = t[k] - (k ? t[k - 1] : 0.0);
+        if (!(span > 0.0)) continue;
+        // the set-up kernel's rule (interval_rule)
+        const double c = std::fmin(std::fmax(1.0, std::ceil(span / dt - 1e-9)), 2e9);
+        steps += (long long)c;
+        if (span / c > kMaxSplitStep) steps_long += (long long)c;
+    }
+    return mostly_long(steps_long, steps);
 }
 
 double constriction_kappa(double c1, double c2)
@@ -464,22 +480,22 @@ int ensure_swarm(iod_problem *p, int m, int trace_needed)
 // cycles a step for 16 particles and one warp of single threads 1,570 for 32).
 bool quads_pay(const iod_problem *p, int m)
 {
-    return p->opt.integrator == IOD_RK4 && p->opt.dynamics == IOD_CR3BP && p->opt.precision == IOD_FP64 &&
-           p->opt.threads_per_particle == 0 && 4LL * m <= 32LL * 4 * sm_count();
+    return !p->fp64_all && p->opt.integrator == IOD_RK4 && p->opt.dynamics == IOD_CR3BP &&
+           p->opt.precision == IOD_FP64 && p->opt.threads_per_particle == 0 && 4LL * m <= 32LL * 4 * sm_count();
 }
 
 // Threads per particle for a swarm of m: two (the lane-pair kernels) or four (quads) for FP64
 // circular swarms, when asked or automatically for small ones.  DOPRI5: 1.05x faster at
 // 1,024 and 4,096 particles, 0.97x at 9,728, 0.56x at 65,536, so pairs up to half the FP64
-// sub-partitions' lanes.  RK4: pairs for the swarms that keep the FP64 step (1.17x), quads
-// for the split step; a request for two threads runs its one-thread kernels, whose results
+// sub-partitions' lanes.  RK4: by FP64 steps pairs while they fit one warp per sub-partition
+// (1.17x faster up to 4,096 particles, 1.09x at 8,192, 0.72x at 16,384), quads for the split step; a request for two threads runs its one-thread kernels, whose results
 // are the same.
 int pick_tpp(const iod_problem *p, int m)
 {
     const int asked = p->opt.threads_per_particle;
     if (asked == 1 || p->opt.precision != IOD_FP64 || p->opt.dynamics != IOD_CR3BP) return 1;
     if (p->opt.integrator == IOD_DOPRI5) return asked == 2 || 4LL * m <= 32LL * 4 * sm_count() ? 2 : 1;
-    if (p->fp64_steps(m)) return 2;
+    if (p->fp64_steps(m)) return asked == 2 || 2LL * m <= 32LL * 4 * sm_count() ? 2 : 1;
     return quads_pay(p, m) ? 4 : 1;
 }
 
@@ -773,6 +789,7 @@ int iod_create_ranged(double mu, const double chief_state[6], int n_obs, const d
         iod::cone_frame(obs_angles[0], obs_angles[1], sigma[0], sigma[1], o.cone_sigmas, o.cone_rho_min,
                         o.cone_rho_max, p->cone);
     cudaGetDevice(&p->device);
+    p->fp64_all = o.integrator == IOD_RK4 && o.dynamics == IOD_CR3BP && iod::long_steps(obs_times, n_obs, o.dt);
 
     auto bail = [&](int code) {
         delete p;
@@ -802,7 +819,7 @@ int iod_create_ranged(double mu, const double chief_state[6], int n_obs, const d
     const KParams P = p->params();
     e = iod::launch_setup(P, o.vmax_frac, sigma[0], sigma[1], o.sigma_range, p->d_chief(), p->d_rc(),
                           p->d_ns(), p->d_h(), p->d_cst(), p->d_gb(), p->d_ep(), nullptr, p->d_rc64(), chief_cs);
-    p->have_rc64 = chief_cs != nullptr;
+    p->have_rc64 = chief_cs != nullptr || p->fp64_all;
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return bail(cuda_fail(e, "set-up kernel"));
     GBest gb;

@@ -57,7 +57,8 @@ struct Layout {
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-Layout layout(int K, int m, int n_tiles, int trace_cap, long long steps_bound, bool mixed, bool refine)
+Layout layout(int K, int m, int n_tiles, int trace_cap, long long steps_bound, bool mixed, bool refine,
+              bool fp64)
 {
     Layout L{};
     size_t o = 0;
@@ -88,11 +89,11 @@ Layout layout(int K, int m, int n_tiles, int trace_cap, long long steps_bound, b
         L.lm = o;
         o = up256(o + sizeof(double) * (kLmVecs * 2 * (size_t)K + kLmTail));
     }
-    // the split residuals' table and, for small swarms and refinements, the chief's positions
-    // by FP64 steps
+    // the split residuals' table and, for requests on FP64 steps and refinements, the chief's
+    // positions by FP64 steps
     L.ep = o;
     o = up256(o + kEpochBytes * (size_t)K);
-    if (m < kFp64Swarm || refine) {
+    if (fp64 || refine) {
         L.rc64 = o;
         o = up256(o + 3 * sizeof(double) * (size_t)K);
     }
@@ -167,11 +168,17 @@ struct iod_batch {
     bool mixed() const { return opt.precision == IOD_MIXED; }
     int trace_cap_for(const Req &r) const { return opt.record_trace ? r.iters + 2 : 0; }
 
+    // whether a request takes FP64 steps (kFp64Swarm, kMaxSplitStep)
+    bool fp64_steps(const Req &r) const
+    {
+        return r.m < kFp64Swarm || long_steps(r.t.data(), (int)r.t.size(), dt_of(r.m));
+    }
+
     size_t bytes_for(const Req &r) const
     {
         const int nt = (r.m + cls_block[class_of(r.m)] - 1) / cls_block[class_of(r.m)];
         return layout((int)r.t.size(), r.m, nt, trace_cap_for(r), steps_bound(r.t, dt_of(r.m)), mixed(),
-                      opt.refine_iters > 0).total;
+                      opt.refine_iters > 0, fp64_steps(r)).total;
     }
 
     void drop_graph()
@@ -225,7 +232,8 @@ int admit(iod_batch *b)
         S.trace_cap = b->trace_cap_for(r);
         S.steps_bound = steps_bound(r.t, b->dt_of(r.m));
         const int K = (int)r.t.size();
-        const Layout L = layout(K, r.m, S.n_tiles, S.trace_cap, S.steps_bound, b->mixed(), b->opt.refine_iters > 0);
+        const Layout L = layout(K, r.m, S.n_tiles, S.trace_cap, S.steps_bound, b->mixed(), b->opt.refine_iters > 0,
+                                b->fp64_steps(r));
         int rc = dev_alloc(S.buf, L.total);
         if (rc) {
             b->free_slots.push_back(si);
@@ -306,7 +314,7 @@ int admit(iod_batch *b)
         P.rng = nullptr;
         P.rc = obs + 4 * K;
         P.ep = (const ff::Epoch *)(base + L.ep);
-        P.fp64 = r.m < kFp64Swarm;
+        P.fp64 = b->fp64_steps(r);
         P.rc64 = P.fp64 || b->opt.refine_iters > 0 ? (const double *)(base + L.rc64) : nullptr;
         P.h = obs + 7 * K;
         P.nsteps = (const int *)(obs + 8 * K);

@@ -18,6 +18,7 @@ namespace iod {
 using namespace dev;
 
 static_assert(sizeof(ff::Epoch) == kEpochBytes, "Epoch table");
+static_assert(kMaxSplitStep == ff::kMaxStep, "longest split step");
 
 namespace {
 
@@ -43,13 +44,14 @@ struct ObsView {
     const ff::Epoch *ep;     // split residuals' table (global memory); null: FP64 residuals
 };
 
-// Propagate s with fixed-step FP64 RK4 through all epochs (circular problem); f(k, s) at
-// each t_k.
+// Propagate s with fixed-step FP64 RK4 in the circular problem over the intervals ending at
+// epochs ka..kb-1 (s is the state at t_{ka-1}, or at t = 0 for ka = 0); f(k, s) at each t_k.
 template <class F>
-__device__ __forceinline__ long long propagate_rk4_fp64(const Dyn &D, double s[6], const ObsView &O, F &&f)
+__device__ __forceinline__ long long propagate_fp64_epochs(const Dyn &D, double s[6], const ObsView &O, int ka, int kb,
+                                                           F &&f)
 {
     long long steps = 0;
-    for (int k = 0; k < O.n; ++k) {
+    for (int k = ka; k < kb; ++k) {
         const int n = O.ns[k];
         const RkH C = rk_h(O.h[k]);
         for (int j = 0; j < n; ++j) rk4_step(D, C, s);
@@ -59,9 +61,7 @@ __device__ __forceinline__ long long propagate_rk4_fp64(const Dyn &D, double s[6
     return steps;
 }
 
-// Propagate s (FP64) with fixed-step RK4 in the elliptic problem over the intervals ending
-// at epochs ka..kb-1 (s is the state at t_{ka-1}, or at t = 0 for ka = 0); f(k, s) at each
-// t_k.
+// The same in the elliptic problem.
 template <class F>
 __device__ __forceinline__ long long propagate_er_epochs(const Dyn &D, double s[6], const ObsView &O, int ka, int kb,
                                                          F &&f)
@@ -90,8 +90,10 @@ __device__ __forceinline__ long long propagate_er_epochs(const Dyn &D, double s[
 }
 
 // The state of a fixed-step propagation in flight: split words for the circular problem
-// (ER = 0; rk4_interval), FP64 for the elliptic one.  kRows values carry it, unchanged,
+// (ER = 0; rk4_interval), FP64 for the elliptic one (1) and the circular one by FP64 steps
+// (kFp64Steps).  kRows values carry it, unchanged,
 // from one warp to the next.
+constexpr int kFp64Steps = 2;
 template <int ER>
 struct RkState {
     static constexpr int kRows = 9;
@@ -172,8 +174,9 @@ struct RkQuad {
     }
 };
 
-template <>
-struct RkState<1> {
+// FP64 steps: the elliptic problem (ER = 1) and the circular problem where it keeps them.
+template <int ER>
+struct RkDouble {
     static constexpr int kRows = 6;
     double s[6];
     __device__ __forceinline__ void begin(const Dyn &, const double x[6])
@@ -194,7 +197,8 @@ struct RkState<1> {
     template <class F>
     __device__ __forceinline__ long long advance(const Dyn &D, const ObsView &O, int ka, int kb, F &&f)
     {
-        return propagate_er_epochs(D, s, O, ka, kb, [&](int k, const double *) { f(k, *this); });
+        auto epoch = [&](int k, const double *) { f(k, *this); };
+        return ER ? propagate_er_epochs(D, s, O, ka, kb, epoch) : propagate_fp64_epochs(D, s, O, ka, kb, epoch);
     }
     __device__ __forceinline__ void get(const Dyn &, double st[6]) const
     {
@@ -208,23 +212,23 @@ struct RkState<1> {
     }
 };
 
-// RK4 propagation through all epochs choosing the dynamics at run time (set-up, propagation
-// and refinement kernels; the swarm kernels choose at compile time).
+template <>
+struct RkState<1> : RkDouble<1> {};
+template <>
+struct RkState<kFp64Steps> : RkDouble<0> {};
+
+// RK4 propagation through all epochs choosing the dynamics at run time (propagation of a
+// caller's states; the swarm kernels choose at compile time).  fp64: by FP64 steps (circular
+// problem).
 template <class F>
-__device__ __forceinline__ long long propagate_rk4_any(const Dyn &D, const double s[6], const ObsView &O, F &&f)
+__device__ __forceinline__ long long propagate_rk4_any(const Dyn &D, bool fp64, double s[6], const ObsView &O, F &&f)
 {
-    double st[6];
-    if (D.er) {
-        RkState<1> R;
-        R.begin(D, s);
-        return R.advance(D, O, 0, O.n, [&](int k, const RkState<1> &r) {
-            r.get(D, st);
-            f(k, st);
-        });
-    }
+    if (D.er) return propagate_er_epochs(D, s, O, 0, O.n, f);
+    if (fp64) return propagate_fp64_epochs(D, s, O, 0, O.n, f);
     RkState<0> R;
     R.begin(D, s);
     return R.advance(D, O, 0, O.n, [&](int k, const RkState<0> &r) {
+        double st[6];
         r.get(D, st);
         f(k, st);
     });
@@ -496,12 +500,12 @@ __device__ __forceinline__ double evaluate(const KParams &P, const Dyn &D, const
     if (INTEG == kRK4 && (ER || !P.fp64)) {
         RkState<ER> R;
         R.begin(D, x);
-        steps += R.advance(D, O, 0, O.n, [&](int k, const RkState<ER> &r) { r.add_cost(D, W, O, k, J); });
+        steps += R.advance(D, O, 0, O.n, [&](int k, const auto &r) { r.add_cost(D, W, O, k, J); });
     } else if (INTEG == kRK4) {
         double s[6];
 #pragma unroll
         for (int d = 0; d < 6; ++d) s[d] = x[d];
-        steps += propagate_rk4_fp64(D, s, O, epoch);
+        steps += propagate_fp64_epochs(D, s, O, 0, O.n, epoch);
     } else {
         double s[6];
 #pragma unroll
@@ -884,9 +888,10 @@ __device__ void setup_intervals(const KParams &P, int *nsteps, double *hs, int t
 }
 
 // Problem set-up, one warp, all lanes alike (after setup_intervals): constants and the chief's
-// positions at
-// the epochs, propagated as the particles are (the rounding that both share cancels in
-// the line of sight).  Returns the number of RK4 steps per propagation.
+// positions at the epochs, propagated as the particles are (the rounding that both share
+// cancels in the line of sight); by FP64 steps (FP64 and P.fp64) in setup_steps instead.
+// Returns the number of RK4 steps per propagation.
+template <int FP64>
 __device__ long long setup_body(const KParams &P, double vmax_frac, double sig_ra, double sig_dec,
                                 double sig_rng, const double *__restrict__ chief, double *rc,
                                 int *nsteps, double *hs, Consts *cst, GBest *gb, ff::Epoch *ep)
@@ -919,7 +924,8 @@ __device__ long long setup_body(const KParams &P, double vmax_frac, double sig_r
         ok = ok && isfinite(st[0]) && isfinite(st[1]) && isfinite(st[2]);
     };
     bool dp_ok = true;
-    if (P.integrator == kRK4 && !D.er) {
+    if (FP64 && P.fp64) {
+    } else if (P.integrator == kRK4 && !D.er) {
         RkQuad R;
         R.begin(D, s);
         R.advance(D, O, [&](int k, const RkState<0> &r) {
@@ -949,6 +955,18 @@ __device__ long long setup_body(const KParams &P, double vmax_frac, double sig_r
     return S;
 }
 
+// The chief's positions by FP64 steps as the problem's own (fp64), spread over threads.
+__device__ void setup_take_fp64(const KParams &P, const double *rc64, double *rc, GBest *gb, int tid, int n)
+{
+    for (int i = tid; i < 3 * P.n_obs; i += n) {
+        const double v = rc64[i];
+        rc[i] = v;
+        if (!isfinite(v)) atomicOr(&gb->status, (int)kStatusChiefDiverged);
+    }
+}
+
+// FP64 = 1: for a problem on FP64 steps (P.fp64).
+template <int FP64>
 __global__ void setup_kernel(KParams P, double vmax_frac, double sig_ra, double sig_dec,
                              double sig_rng, const double *__restrict__ chief, double *rc,
                              int *nsteps, double *hs, Consts *cst, GBest *gb, ff::Epoch *ep, double *rc64,
@@ -957,10 +975,13 @@ __global__ void setup_kernel(KParams P, double vmax_frac, double sig_ra, double 
     if (blockIdx.x != 0) return;
     setup_intervals(P, nsteps, hs, threadIdx.x, blockDim.x);
     __syncthreads();
-    if (threadIdx.x < 32) setup_body(P, vmax_frac, sig_ra, sig_dec, sig_rng, chief, rc, nsteps, hs, cst, gb, ep);
+    if (threadIdx.x < 32) setup_body<FP64>(P, vmax_frac, sig_ra, sig_dec, sig_rng, chief, rc, nsteps, hs, cst, gb, ep);
     if (threadIdx.x >= 64) setup_angles(P, ep, threadIdx.x - 64, blockDim.x - 64);
     // the second warp, beside the first
-    if (cs && threadIdx.x >= 32 && threadIdx.x < 34) setup_steps(P, chief, rc64, cs, threadIdx.x - 32);
+    if ((cs || FP64) && threadIdx.x >= 32 && threadIdx.x < 34) setup_steps(P, chief, rc64, cs, threadIdx.x - 32);
+    if (!FP64) return;
+    __syncthreads();
+    setup_take_fp64(P, rc64, rc, gb, threadIdx.x, blockDim.x);
 }
 
 __global__ void setup_fp64_kernel(KParams P, const double *__restrict__ chief, double *rc64)
@@ -1140,7 +1161,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) propagate_kernel(KParams P, co
         for (int d = 0; d < 6; ++d) out[((size_t)k * 6 + d) * m + i] = st[d];
     };
     if (INTEG == kRK4) {
-        propagate_rk4_any(D, s, O, store);
+        propagate_rk4_any(D, P.fp64, s, O, store);
     } else {
         bool ok;
         if (D.er)
@@ -2148,7 +2169,7 @@ __global__ void __launch_bounds__(32 * kBalancedMaxWarpsPerSm, 1) iter_kernel_ba
                 }
                 R.begin(D, x);
             }
-            steps += R.advance(D, O, ea, eb, [&](int k, const RkState<ER> &r) { r.add_cost(D, W, O, k, J); });
+            steps += R.advance(D, O, ea, eb, [&](int k, const auto &r) { r.add_cost(D, W, O, k, J); });
         }
         if (out) {
             double *h = S->hand + (size_t)wj * kHandRows * 32;
@@ -2636,7 +2657,7 @@ __global__ void batch_setup_kernel(BatchSlot *slots, const int *__restrict__ ids
     setup_intervals(B.P, B.ns_w, B.h_w, threadIdx.x, blockDim.x);
     __syncthreads();
     if (threadIdx.x < 32) {
-        const long long S = setup_body(B.P, B.vmax_frac, B.sig_ra, B.sig_dec, B.sig_rng, B.chief, B.rc_w, B.ns_w,
+        const long long S = setup_body<1>(B.P, B.vmax_frac, B.sig_ra, B.sig_dec, B.sig_rng, B.chief, B.rc_w, B.ns_w,
                                        B.h_w, B.cst_w, B.P.gb, B.ep_w);
         if (threadIdx.x == 0) B.P.total_steps = S;
     }
@@ -2647,6 +2668,7 @@ __global__ void batch_setup_kernel(BatchSlot *slots, const int *__restrict__ ids
     if ((mixed || B.rc64_w) && threadIdx.x >= 32 && threadIdx.x < 34)
         setup_steps(B.P, B.chief, B.rc64_w, mixed ? B.cs_w : nullptr, threadIdx.x - 32);
     __syncthreads();
+    if (B.P.fp64) setup_take_fp64(B.P, B.rc64_w, B.rc_w, B.P.gb, threadIdx.x, blockDim.x);
     if (B.n_mixed >= 0) setup_mixed_body(B.P, B.mix_w, B.cs_w, B.od_w, B.ct_w, threadIdx.x, blockDim.x);
 }
 
@@ -2984,7 +3006,7 @@ __device__ bool lm_residuals(const Dyn &D, const ObsView &O, const double x[6], 
     if (D.er)
         propagate_er_epochs(D, s, O, 0, O.n, epoch);
     else
-        propagate_rk4_fp64(D, s, O, epoch);
+        propagate_fp64_epochs(D, s, O, 0, O.n, epoch);
     cost = (ok && isfinite(c)) ? c : CUDART_INF;
     return ok;
 }
@@ -3410,8 +3432,12 @@ cudaError_t launch_setup(const KParams &P, double vmax_frac, double sigma_ra, do
                          double *h_out, Consts *cst_out, GBest *gb, ff::Epoch *ep, cudaStream_t st, double *rc64,
                          double *chief_cs)
 {
-    setup_kernel<<<1, 128, 0, st>>>(P, vmax_frac, sigma_ra, sigma_dec, sigma_rng, chief, rc_out,
-                                   nsteps_out, h_out, cst_out, gb, ep, rc64, chief_cs);
+    if (P.fp64)
+        setup_kernel<1><<<1, 128, 0, st>>>(P, vmax_frac, sigma_ra, sigma_dec, sigma_rng, chief, rc_out, nsteps_out,
+                                           h_out, cst_out, gb, ep, rc64, chief_cs);
+    else
+        setup_kernel<0><<<1, 128, 0, st>>>(P, vmax_frac, sigma_ra, sigma_dec, sigma_rng, chief, rc_out, nsteps_out,
+                                           h_out, cst_out, gb, ep, rc64, chief_cs);
     return cudaGetLastError();
 }
 
@@ -3721,6 +3747,13 @@ cudaError_t launch_iter_balanced(const KParams &P, int mode, int nsm, int wps, c
         if (mode == 2) IOD_BAL_DP(2); else if (mode == 1) IOD_BAL_DP(1); else IOD_BAL_DP(0);
     } else if (P.dynamics) {
         if (mode == 2) IOD_BAL(2, 1); else if (mode == 1) IOD_BAL(1, 1); else IOD_BAL(0, 1);
+    } else if (P.fp64) {
+        if (mode == 2)
+            IOD_BAL(2, kFp64Steps);
+        else if (mode == 1)
+            IOD_BAL(1, kFp64Steps);
+        else
+            IOD_BAL(0, kFp64Steps);
     } else {
         if (mode == 2) IOD_BAL(2, 0); else if (mode == 1) IOD_BAL(1, 0); else IOD_BAL(0, 0);
     }
@@ -3835,6 +3868,13 @@ score_noalloc_kernel(double mu, int K, const double *__restrict__ obs, double si
         rcz[k] = obs[5 * K + k];
         interval_rule(k ? obs[k - 1] : 0.0, obs[k], dt, ns[k], h[k]);
     }
+    __shared__ int s_steps, s_long;
+    if (threadIdx.x == 0) s_steps = s_long = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        atomicAdd(&s_steps, ns[k]);
+        if (h[k] > kMaxSplitStep) atomicAdd(&s_long, ns[k]);
+    }
     __syncthreads();
     const ObsView O{ra, dec, nullptr, rcx, rcy, rcz, t, h, ns, K, nullptr};
     const Dyn D{mu, 1.0 - mu};
@@ -3847,6 +3887,7 @@ score_noalloc_kernel(double mu, int K, const double *__restrict__ obs, double si
     KParams P{};
     P.mu = mu;
     P.n_obs = K;
+    P.fp64 = mostly_long(s_long, s_steps);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double x[6] = {0, 0, 0, 0, 0, 0};
     double J = CUDART_INF;
