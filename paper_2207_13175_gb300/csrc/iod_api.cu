@@ -417,16 +417,31 @@ int check_shard(const iod_problem *p, int m)
     return IOD_OK;
 }
 
-// The chief's positions by FP64 steps (circular problem), formed when first asked for.
+// The chief's positions by FP64 steps (circular problem), formed when first asked for: on the
+// problem's stream, or, while that is being captured, at once on a stream of its own (a
+// graph would form them again at every replay).
 int ensure_rc64(iod_problem *p)
 {
     if (p->have_rc64 || p->opt.dynamics == IOD_ER3BP) return IOD_OK;
-    cudaError_t e = iod::launch_setup_fp64(p->params(), p->d_chief(), p->d_rc64(), p->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "set-up kernel");
-    // (a captured launch writes the table when the graph runs, which it may never do)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     IOD_CUDA(cudaStreamIsCapturing(p->stream, &cap), "cudaStreamIsCapturing");
-    p->have_rc64 = cap == cudaStreamCaptureStatusNone;
+    cudaError_t e;
+    if (cap == cudaStreamCaptureStatusNone) {
+        e = iod::launch_setup_fp64(p->params(), p->d_chief(), p->d_rc64(), p->stream);
+    } else {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        IOD_CUDA(cudaThreadExchangeStreamCaptureMode(&mode), "cudaThreadExchangeStreamCaptureMode");
+        cudaStream_t st = nullptr;
+        e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e == cudaSuccess) {
+            e = iod::launch_setup_fp64(p->params(), p->d_chief(), p->d_rc64(), st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            cudaStreamDestroy(st);
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "set-up kernel");
+    p->have_rc64 = true;
     return IOD_OK;
 }
 
