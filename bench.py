@@ -43,8 +43,8 @@ FLOP_PER_MOVE = 50
 # x 2070 MHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # FP64 form: the circular problem's RK4 step runs in sums of FP32 words, 259 single and 369
-# paired FP32 instructions (44 and 90 of them FMAs), so its roofline is the FP32 pipe's
-SPLIT_OPS_PER_STEP = 259 + 44 + 2 * (369 + 90)
+# paired FP32 instructions (44 and 93 of them FMAs), so its roofline is the FP32 pipe's
+SPLIT_OPS_PER_STEP = 259 + 44 + 2 * (369 + 93)
 # mixed form: its roofline counts the method's work, the same algorithmic operations as
 # the FP64 form (FLOP_PER_STEP, FLOP_PER_EPOCH, FLOP_PER_MOVE), executed in FP32 against
 # the FP32 peak (152 SMs x 128 FP32 FMA/clk x 2 flop x 2070 MHz).  Beside it, the FP32
@@ -68,8 +68,8 @@ FLOP_PER_DP_EPOCH = 52 + 6 * 13 + FLOP_PER_EPOCH
 # full 65,536 particles (10.64 MB)
 TRAFFIC_FP64_65K = 2590464 * 4
 # the balanced FP64 iteration (the automatic choice for 65,536 particles on 152 SMs),
-# mean of five full-size launches of the current kernel (10.29 MB read, 2 KB written)
-TRAFFIC_FP64_BAL_65K = 10296781
+# mean of five full-size launches of the current kernel (10.37 MB read, 3 KB written)
+TRAFFIC_FP64_BAL_65K = 10373120
 TRAFFIC_MIXED_65K = 10640000
 # the balanced mixed iteration (the automatic choice at 65,536 particles on 152 SMs),
 # mean of three full-size launches of the current kernel (10.77 MB read, 0.2 KB written)

@@ -76,10 +76,22 @@ typedef struct iod_options {
     double rtol, atol;       /* DOPRI5 tolerances.  Default 1e-12, 1e-12 */
     double h0;               /* DOPRI5 first step (TU).  Default 1e-3 */
     long long max_steps;     /* DOPRI5 attempts per propagation before J = +inf.  Default 1e7 */
-    int precision;           /* IOD_FP64 (default; the circular problem's RK4 steps are taken in
-                                unevaluated sums of FP32 words, 48 to 72 bits, wherever
-                                that is at least as exact as an FP64 step; swarms below
-                                256 particles and the refinement in FP64) or IOD_MIXED (RK4 only): iterations are
+    int precision;           /* IOD_FP64 (default) or IOD_MIXED (RK4 only).
+                                IOD_FP64: the circular problem's RK4 steps up to 2.1e-3 TU are
+                                taken in unevaluated sums of FP32 words (48 to 72 bits)
+                                where that errs no more than an FP64 step would (root mean
+                                square position errors at most 1.05 times, 1.3 times on
+                                orbits that stay 0.75 to 0.9 from the larger primary for a
+                                week at steps above 1e-3; far less about the smaller one);
+                                nearer to the primaries, for longer steps, in swarms
+                                below 256 particles and in the refinement FP64 steps are.
+                                A swarm's costs are iod_eval's, bit for bit, from 256
+                                particles on; below, they differ by the FP64 steps'
+                                rounding.  Angle residuals of every FP64 form are formed in
+                                two FP32 words (1.4e-15 rad, root mean square) as long as
+                                the positions' own rounding is the larger error, else (lines
+                                of sight above sqrt(1 + n)/32 LU after n steps) in FP64.
+                                IOD_MIXED: iterations are
                                 propagated in FP32 as offsets from the chief until the last
                                 fp64_last_iters, then every personal best is re-evaluated in
                                 FP64 and the remaining iterations run in FP64 (iod_run with
@@ -128,10 +140,11 @@ typedef struct iod_options {
                                 block d; dimension 0 keeps the shared pair) */
     int threads_per_particle;/* 1: one thread per particle; 2: a lane pair per particle, each
                                 lane evaluating one primary's attraction (FP64 circular
-                                problems with DOPRI5, or RK4 swarms below 256 particles;
-                                other RK4 swarms run as with 1; results identical to 1); 0
-                                (default): chosen by integrator and swarm size, up to four
-                                lanes per particle (results identical to 1) */
+                                problems with DOPRI5, or RK4 by FP64 steps: swarms below 256
+                                particles or steps above 2.1e-3 TU; other RK4 swarms run
+                                as with 1, in the grid form); 0 (default): chosen by
+                                integrator and swarm size, up to four lanes per particle.
+                                Results are identical in all forms */
     /* Dynamics.  IOD_CR3BP (default): Eqs. 1-3.  IOD_ER3BP: the elliptic restricted
      * problem, named by the paper as future work, in Szebehely's pulsating rotating frame
      * with the true anomaly f as independent variable: x'' - 2y' = d(omega)/dx,
@@ -165,7 +178,9 @@ typedef struct iod_options {
      * best by Levenberg-Marquardt (Sec. "Local Minimization", Eqs. 14-16), FP64, at most
      * refine_iters iterations, residuals of the cost form (CHI2: the 2K weighted angle
      * residuals; QUARTIC: the K per-epoch chi-squares).  The request's result is then the
-     * refined state and cost, with the swarm's own best beside it (pso_state, pso_cost).
+     * refined state and cost as iod_refine gives them (the swarm's best itself, with its
+     * recorded cost, if nothing better was found), with the swarm's own best beside it
+     * (pso_state, pso_cost).
      * 0 (default): no refinement. */
     int refine_iters;
     /* Sharded swarms (single problems, IOD_FP64, tol_tau = 0): this problem holds particles

@@ -1174,7 +1174,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) propagate_kernel(KParams P, co
     }
 }
 
-// The same of the circular problem on quads of lanes (m up to quad_swarm()): quads past the
+// The same of the circular problem on quads of lanes (quads_pay in iod_api.cu): quads past the
 // end follow state 0.
 __global__ void __launch_bounds__(kQuadBlock, 1) eval_quad_kernel(KParams P, const double *__restrict__ X, int m,
                                                                double *__restrict__ Jout)
@@ -2873,8 +2873,8 @@ __global__ void wq_seed_kernel(BatchSlot *slots, int n_slots, WorkQueue *q, int2
 // action publishes its next action at once (until the device-time budget is spent),
 // so problems advance independently.  Blocks leave when no problem has work left in
 // this launch, or when one wait has lasted kWqWaitLimitNs (status kWqTimeout).
-// MINB resident blocks of 256 threads per SM at least: 2 (128 registers, no spills) keeps
-// each block's chains fastest, the latency form for a few requests; 3 (80 registers, the
+// MINB resident blocks of 256 threads per SM at least: 2 (128 registers, about 360 bytes
+// spilled) keeps each block's chains fastest, the latency form for a few requests; 3 (80 registers, the
 // bodies spilling about a kilobyte per thread to local memory) runs a full batch 5%
 // faster (64 registers: 16% slower), the throughput form.
 template <int MINB>

@@ -1,21 +1,26 @@
-// Host build of the split RK4 step (iod_ff.cuh): root mean square position error over that
-// of a plain FP64 RK4, circular orbits about a primary, RK4 in long double as reference.
-// Arguments: groups of (moon, mu, r, h, T); prints one ratio per group.
+// Host build of the split RK4 step (iod_ff.cuh) and residuals (iod_ff_cost.cuh).  Prints, for
+// groups of arguments (moon, mu, r, h, T), the root mean square position error over that of a
+// plain FP64 RK4 (circular orbits about a primary, RK4 in long double as reference); the
+// number of state components that words change; and the residuals' root mean square and
+// largest error in rad, below 0.1 rad and over the circle.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <random>
 
-// stands for the hardware's estimate of x^(-1/2): the root with a relative error up to 2^-23
-static float rsqrt_estimate(float x)
+// stand for the hardware's estimates: x^(-1/2) and 1/x with relative errors up to 2^-23
+static double off()
 {
     static unsigned int state = 12345;
     state = state * 1664525u + 1013904223u;
-    return (float)((1.0 / std::sqrt((double)x)) * (1.0 + ((state >> 8) / 8388608.0 - 1.0) * 0x1p-23));
+    return 1.0 + ((state >> 8) / 8388608.0 - 1.0) * 0x1p-23;
 }
+static float rsqrt_estimate(float x) { return (float)(1.0 / std::sqrt((double)x) * off()); }
+static float rcp_estimate(float x) { return (float)(1.0 / (double)x * off()); }
 #define IOD_RSQRT_EST(x) rsqrt_estimate(x)
-#include "iod_ff.cuh"
+#define IOD_RCP_EST(x) rcp_estimate(x)
+#include "iod_ff_cost.cuh"
 
 using namespace iod::ff;
 typedef long double Ref;
@@ -137,11 +142,50 @@ static int changed()
     return bad;
 }
 
+// residuals of lines of sight within `width` of the observed angles, elevations up to 1.4
+static void residual_errors(double width, double &rms, double &most)
+{
+    const Ref pi = 3.14159265358979323846264338327950288L;
+    std::mt19937_64 rng(2);
+    auto u = [&]() { return (double)(rng() >> 11) * 0x1p-52 - 1.0; };
+    int n = 0;
+    rms = most = 0;
+    for (int i = 0; i < 200000; ++i) {
+        const double ra = 3.1 * u(), dec = 1.3 * u(), a = ra + width * u(), el = dec + width * u();
+        if (std::fabs(el) > 1.4) continue;
+        const double ca = std::cos(ra), sa = std::sin(ra), cb = std::cos(dec), sb = std::sin(dec);
+        Epoch E{};
+        E.ok = 1;
+        E.far2 = 1.0f;
+        E.ka = mk2((float)ca, (float)sa);
+        E.kal = mk2((float)(ca - (double)E.ka.x), (float)(sa - (double)E.ka.y));
+        E.kb = mk2((float)cb, (float)sb);
+        E.kbl = mk2((float)(cb - (double)E.kb.x), (float)(sb - (double)E.kb.y));
+        const double x = 0.01 * std::cos(el) * std::cos(a), y = 0.01 * std::cos(el) * std::sin(a), z = 0.01 * std::sin(el);
+        const float2 h = mk2((float)x, (float)y), l = mk2((float)(x - (double)h.x), (float)(y - (double)h.y));
+        float2 bh, bl;
+        float rh, rl;
+        if (!residuals(E, h, l, (float)z, (float)(z - (double)(float)z), bh, bl, rh, rl)) continue;
+        const Ref A = std::fabs(std::remainder((Ref)ra - std::atan2((Ref)y, (Ref)x), 2 * pi));
+        const Ref B = std::fabs((Ref)dec - std::asin((Ref)z / std::sqrt((Ref)x * x + (Ref)y * y + (Ref)z * z)));
+        const double e = (double)((Ref)bh.x + bl.x - A), f = (double)((Ref)bh.y + bl.y - B);
+        rms += e * e + f * f;
+        most = std::max(most, std::max(std::fabs(e), std::fabs(f)));
+        n += 2;
+    }
+    rms = std::sqrt(rms / n);
+}
+
 int main(int argc, char **argv)
 {
     for (int i = 1; i + 4 < argc; i += 5)
         std::printf("%.4f\n", ratio(std::atoi(argv[i]), std::atof(argv[i + 1]), std::atof(argv[i + 2]),
                                     std::atof(argv[i + 3]), std::atof(argv[i + 4])));
     std::printf("%d\n", changed());
+    for (double width : {0.1, 3.1}) {
+        double rms, most;
+        residual_errors(width, rms, most);
+        std::printf("%.3e\n%.3e\n", rms, most);
+    }
     return 0;
 }

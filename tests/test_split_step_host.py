@@ -1,6 +1,7 @@
 """The split RK4 step's host build (tests/split_step_host.cpp): circular orbits over steps of
 1e-5 to 2e-3, distances from 0.08 of the Earth and 0.002 of the Moon, several mass parameters,
-are no less exact than plain FP64 steps; and states come back from their words unchanged."""
+are no less exact than plain FP64 steps; states come back from their words unchanged; and the
+split residuals err by what the header states."""
 import os
 import shutil
 import subprocess
@@ -41,3 +42,11 @@ def test_no_less_exact_than_fp64(result):
 
 def test_states_come_back_from_words(result):
     assert result[len(CASES)] == "0"
+
+
+def test_residual_errors(result):
+    rms, most, rms_all, most_all = map(float, result[len(CASES) + 1:])
+    # each residual passes about ten operations on second words, 2^-49 of angles up to pi/2
+    # (below 0.1 rad) or pi: 10^0.5 2^-49 pi/2 / sqrt(3) root mean square, ten of them at most
+    assert rms <= 5.1e-15 and rms_all <= 1.1e-14, (rms, rms_all)
+    assert most <= 2.8e-14 and most_all <= 5.6e-14, (most, most_all)
