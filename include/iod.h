@@ -80,9 +80,9 @@ typedef struct iod_options {
                                 IOD_FP64: the circular problem's RK4 steps up to 2.1e-3 TU are
                                 taken in unevaluated sums of FP32 words (48 to 72 bits)
                                 where that errs no more than an FP64 step would (root mean
-                                square position errors at most 1.05 times, 1.3 times on
-                                orbits that stay 0.75 to 0.9 from the larger primary for a
-                                week at steps above 1e-3; far less about the smaller one);
+                                square position errors at most 1.05 times, 1.35 times on
+                                orbits that stay 0.75 to 1 from the larger primary for a
+                                week at steps from 1e-3; far less about the smaller one);
                                 nearer to the primaries, for longer steps, in swarms
                                 below 256 particles and in the refinement FP64 steps are.
                                 A swarm's costs are iod_eval's, bit for bit, from 256
